@@ -1,0 +1,110 @@
+"""The float64 functions of the kernels' law header, compiled for the host with models of the fast float32 functions
+that they start from (tests/host/float64_functions.cpp), against 80-bit arithmetic: every result has to hold for every
+error that CUDA documents for those starts."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+TILTS = [(a, b) for a in (-1.0, 0.0, 1.0) for b in (-1.0, 0.0, 1.0)]
+LD = np.longdouble
+
+
+def _cuda_include():
+    nvcc = shutil.which(os.environ.get("NVCC", "nvcc")) or "/usr/local/cuda/bin/nvcc"
+    return os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "float64_functions.so")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-w", "-shared", "-fPIC", "-I" + _cuda_include(),
+                    "-I" + os.path.join(ROOT, "include"), "-I" + os.path.join(ROOT, "paper_2004_08503_gb300", "csrc"),
+                    os.path.join(HERE, "host", "float64_functions.cpp"), "-o", so], check=True)
+    return ctypes.CDLL(so)
+
+
+def _p(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def _tilt(lib, t):
+    lib.set_tilt(ctypes.c_double(t[0]), ctypes.c_double(t[1]))
+
+
+def _psi(u, K, gamma):
+    u = u.astype(LD)
+    return u[:, 3] - (u[:, 1] ** 2 + u[:, 2] ** 2) / (2 * u[:, 0]) - K.astype(LD) * u[:, 0] ** LD(gamma)
+
+
+def _psi_at(u, w, s, K, gamma):
+    return _psi(u.astype(LD) + s * w.astype(LD), K, gamma)
+
+
+def _states(rng, n, gamma, decades):
+    """States of all densities, Mach numbers up to 3, K just below the state's own sigma."""
+    rho = 10.0 ** rng.uniform(-decades, decades, n)
+    rhoe = rho * 10.0 ** rng.uniform(-1, 1, n)
+    c = np.sqrt(gamma * (gamma - 1.0) * rhoe / rho)
+    v = c[:, None] * rng.uniform(-2, 2, (n, 2))
+    u = np.column_stack([rho, rho[:, None] * v, rhoe + 0.5 * rho * np.sum(v * v, axis=1)])
+    K = (_psi(u, np.zeros(n), gamma) * (1 - 10.0 ** rng.uniform(-8, -2, n)) / rho.astype(LD) ** LD(gamma)).astype(float)
+    w = u * 10.0 ** rng.uniform(-7, -1, (n, 1)) * rng.uniform(-1, 1, (n, 4))
+    return u, K, w
+
+
+def _screen(lib, gamma, u, K, w, sc, tcap):
+    out = np.empty(len(u), np.int32)
+    lib.screen(len(u), ctypes.c_double(gamma), _p(u), _p(K), _p(w), ctypes.c_double(sc), ctypes.c_double(tcap), _p(out))
+    return out.astype(bool)
+
+
+@pytest.mark.parametrize("gamma", [1.4, 5.0 / 3.0, 1.1])
+@pytest.mark.parametrize("decades", [1, 4, 12, 17.5])
+def test_screen_passes_no_inadmissible_candidate(lib, gamma, decades):
+    """Candidates with psi_K below zero by 1e-9 to 1e-4 of rho e: none of them may be called certain."""
+    rng = np.random.default_rng(int(10 * decades))
+    u, K, w = _states(rng, 40000, gamma, decades)
+    sc, tcap = 0.37, 0.9
+    target = -(10.0 ** rng.uniform(-9, -4, len(u))) * _psi(u, np.zeros(len(u)), gamma)
+    s = LD(sc) * LD(tcap)
+    for _ in range(2):  # psi is affine in the energy: move the candidate onto its target
+        w[:, 3] += ((target - _psi_at(u, w, s, K, gamma)) / s).astype(float)
+    bad = _psi_at(u, w, s, K, gamma) < 0
+    assert bad.mean() > 0.99
+    for t in TILTS:
+        _tilt(lib, t)
+        undecided = _screen(lib, gamma, u, K, w, sc, tcap)
+        wrong = bad & ~undecided
+        assert not wrong.any(), (t, int(wrong.sum()), float((target[wrong] / _psi(u, np.zeros(len(u)), gamma)[wrong]).min()))
+
+
+def test_screen_decides_clear_candidates(lib):
+    """The screen is worth its cost: candidates with psi_K above zero by 1e-4 of rho E are certain."""
+    rng = np.random.default_rng(3)
+    u, K, w = _states(rng, 20000, 1.4, 12)
+    K, w = 0.9 * K, 1e-3 * w
+    ok = _psi_at(u, w, LD(0.5), K, 1.4) > 1e-4 * u[:, 3]
+    assert ok.mean() > 0.9
+    for t in TILTS:
+        _tilt(lib, t)
+        assert not _screen(lib, 1.4, u, K, w, 1.0, 0.5)[ok].any(), t
+
+
+@pytest.mark.parametrize("gamma", [1.4, 5.0 / 3.0, 1.1])
+def test_sigma_certainly_above_is_certain(lib, gamma):
+    """States with sigma below K by 1e-9 to 1e-3: none may be called certainly above."""
+    rng = np.random.default_rng(4)
+    u, K, _ = _states(rng, 40000, gamma, 17.5)
+    sig = _psi(u, np.zeros(len(u)), gamma) / u[:, 0].astype(LD) ** LD(gamma)
+    K = (sig * (1 + 10.0 ** rng.uniform(-9, -3, len(u)))).astype(float)
+    out = np.empty(len(u), np.int32)
+    for t in TILTS:
+        _tilt(lib, t)
+        lib.certainly_above(len(u), ctypes.c_double(gamma), _p(u), _p(K), _p(out))
+        assert not out.any(), (t, int(out.sum()))
