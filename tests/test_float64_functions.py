@@ -108,3 +108,21 @@ def test_sigma_certainly_above_is_certain(lib, gamma):
         _tilt(lib, t)
         lib.certainly_above(len(u), ctypes.c_double(gamma), _p(u), _p(K), _p(out))
         assert not out.any(), (t, int(out.sum()))
+
+
+def test_minima_and_sign_tests(lib):
+    """The integer forms against fmax, fmin and the comparisons, NaN of both signs, infinities, zeros and denormals among
+    the operands; every result bit for bit but for the sign of a zero and which NaN comes out of two."""
+    rng = np.random.default_rng(5)
+    v = np.concatenate([[0.0, -0.0, 5e-324, -5e-324, 2.2e-308, 1.0, -1.0, 1.0 + 2e-16, 1e308, -1e308, np.inf, -np.inf, np.nan,
+                         -np.nan, np.copysign(np.nan, -1.0)], rng.normal(size=20) * 10.0 ** rng.uniform(-300, 300, 20)])
+    a, b = (np.ascontiguousarray(m.ravel()) for m in np.meshgrid(v, v))
+    out = np.empty((5, a.size))
+    lib.compare_ops(a.size, _p(a), _p(b), _p(out))
+    for got, exp in zip(out, (np.fmax(a, b), np.fmin(a, b), np.fmax(a, 0.0), np.fmin(a, 0.0), (a > 0).astype(float))):
+        np.testing.assert_array_equal(got, exp)
+    a, b = np.where(np.isnan(a), a, np.abs(a)), np.where(np.isnan(b), b, np.abs(b))  # >= +0, or a NaN of either sign
+    out = np.empty((2, a.size))
+    lib.compare_ops_nonneg(a.size, _p(a), _p(b), _p(out))
+    for got, exp in zip(out, (np.fmax(a, b), np.fmin(a, b))):
+        np.testing.assert_array_equal(got, exp)

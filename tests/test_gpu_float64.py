@@ -1,4 +1,5 @@
-"""The float64 path where its cheap forms meet their limits: densities far from 1."""
+"""The float64 path where its cheap forms meet their limits: densities far from 1, nodes
+without a real sound speed."""
 import numpy as np
 import pytest
 
@@ -28,3 +29,25 @@ def test_entropy_minimum_holds_at_every_density(size, gamma):
         sv.close()
         assert d["max_entropy_violation"] <= 1e-12, (amp, d["max_entropy_violation"])
         assert d["max_bound_violation"] <= 1e-12
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("limiter", ["none", "lo"])
+@pytest.mark.parametrize("node", [0, 1, 4])
+def test_negative_pressure_at_a_face_keeps_the_neighbours_speed(node, limiter, precision):
+    """One node (a corner, a face node) with p < 0, as the unlimited scheme can produce: its sound speed is NaN,
+    its faces take the neighbour's finite speed, and the time step and the stage stay finite, in both precisions."""
+    sv = sidp.Solver(law="euler", p=3, nx=7, ny=6, domain=(0.0, 1.4, 0.0, 1.2), bc=("outflow",) * 4, limiter=limiter,
+                     precision=precision)
+    x, y = sv.node_coords()
+    u = waves(x, y, 0.1)
+    i = (2 * 7 + 3) * 16 + node
+    u[3, i] = 0.3 * (u[1, i] ** 2 + u[2, i] ** 2) / u[0, i]
+    v = np.ascontiguousarray(u, dtype=np.float64 if precision == "fp64" else np.float32)
+    sidp.sidp_upload_state(sv.ctx, v.ctypes.data)  # set_state takes admissible states only
+    dt = sv.compute_dt()
+    assert 0.0 < dt < 1.0
+    sv.stage(1, dt)
+    got = sv.get_state(1)
+    sv.close()
+    assert np.all(np.isfinite(got))
