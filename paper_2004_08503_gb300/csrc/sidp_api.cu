@@ -85,7 +85,7 @@ __device__ __forceinline__ void diag_reduce(double* acc, double (*red)[kDiagThre
 
 // Diagnostics of a state in one launch: every block's sums and extremes into `part`, the last block's
 // reduction of them with the clock and the statistics into `out`.  The extremes are taken in the stored
-// type and the masses of a node from a table, so that a node costs 12 float64 operations (its products
+// type and the masses of a node from a table, so that a node costs 14 float64 operations (its products
 // with the mass, its pressure); 60 with float64 minima, products of weights and an IEEE division, and one
 // thread reducing the blocks, took 258 us on any small mesh and 1.9 ms on 16.8M nodes.
 template <typename T, int NC>
@@ -124,7 +124,7 @@ k_diag(const T* __restrict__ u, long long N, int n, double h, const double* __re
       hi[f] = tmax(hi[f], x);
     }
     if constexpr (NC == 4) {
-      const double p = v[3] - 0.5 * (v[1] * v[1] + v[2] * v[2]) * frcp(v[0]);
+      const double p = v[3] - fdiv(0.5 * (v[1] * v[1] + v[2] * v[2]), v[0]);
       if (p == p) pmin = tmin(pmin, p);
     }
   }

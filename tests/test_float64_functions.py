@@ -126,3 +126,33 @@ def test_minima_and_sign_tests(lib):
     lib.compare_ops_nonneg(a.size, _p(a), _p(b), _p(out))
     for got, exp in zip(out, (np.fmax(a, b), np.fmin(a, b))):
         np.testing.assert_array_equal(got, exp)
+
+
+def test_quotients_and_roots_round_like_ieee(lib):
+    """a / b, 1 / b and the root over all exponents: within half an ulp and 1e-5 of the 80-bit value (whose own
+    resolution is 2^-11 ulp) where the result is normal, and the IEEE results for zeros, infinities, NaN, overflow and denormals."""
+    rng = np.random.default_rng(6)
+    n = 100000
+    for decades in (1, 28, 307):
+        a, b = (rng.choice([-1.0, 1.0], n) * rng.uniform(1, 2, n) * 10.0 ** rng.uniform(-decades, decades, n) for _ in range(2))
+        b[: n // 2] = np.abs(b[: n // 2])
+        out = np.empty((3, n))
+        with np.errstate(all="ignore"):
+            exact = [a.astype(LD) / b, 1 / b.astype(LD), np.sqrt(b.astype(LD))]
+            ieee = [a / b, 1 / b, np.sqrt(b)]
+        for t in TILTS[::3]:
+            _tilt(lib, t)
+            lib.quotients(n, _p(a), _p(b), _p(out))
+            for got, x, i in zip(out, exact, ieee):
+                normal = np.isfinite(i) & (np.abs(i) > 1e-290)
+                ulps = np.abs(got[normal] - x[normal]) / np.spacing(np.abs(i[normal]))
+                assert ulps.max() <= 0.5 + 2.0 ** -11 + 1e-5, (decades, t, float(ulps.max()))
+                np.testing.assert_allclose(got[~normal], i[~normal], rtol=0, atol=5e-324)
+    v = np.array([0.0, -0.0, 5e-324, 1e-310, 1e-300, 1e-40, 1.0, -3.0, 1e40, 1e300, np.inf, -np.inf, np.nan])
+    a, b = (np.ascontiguousarray(m.ravel()) for m in np.meshgrid(v, v))
+    out = np.empty((3, a.size))
+    _tilt(lib, (0.0, 0.0))
+    lib.quotients(a.size, _p(a), _p(b), _p(out))
+    with np.errstate(all="ignore"):
+        for got, exp in zip(out, (a / b, 1 / b, np.sqrt(b))):
+            np.testing.assert_array_equal(got, exp)
