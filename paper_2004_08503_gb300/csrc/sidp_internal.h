@@ -32,6 +32,7 @@ struct LawParamsT {
   int pow7;     // inv_e == 7 (gamma = 1.4): powers by products and roots instead of pow
   double gamma_d;  // gamma in float64 (statistics)
   float gamma_f;   // gamma in float32 (the float64 path's screen)
+  float rest_gamma, rest_neg_e, rest_inv_e;  // pow7: (gamma - 7/5, neg_e + 1/7, inv_e - 7) ln 2
 };
 
 template <typename T>
@@ -52,6 +53,11 @@ inline LawParamsT<T> make_law_params(double gamma, const double* beta, const dou
   p.pow7 = (2.0 * g / (g - 1.0) > 7.0 - 1e-12 && 2.0 * g / (g - 1.0) < 7.0 + 1e-12) ? 1 : 0;
   p.gamma_d = g;
   p.gamma_f = (float)g;
+  // the rests exactly: 5 gamma - 7 and 7 neg_e + 1 in one rounding each
+  const double ne = -(g - 1.0) / (2.0 * g), ln2 = 0.69314718055994530942;
+  p.rest_gamma = (float)(std::fma(5.0, g, -7.0) / 5.0 * ln2);
+  p.rest_neg_e = (float)(std::fma(7.0, ne, 1.0) / 7.0 * ln2);
+  p.rest_inv_e = (float)((2.0 * g / (g - 1.0) - 7.0) * ln2);
   return p;
 }
 
