@@ -124,7 +124,7 @@ k_diag(const T* __restrict__ u, long long N, int n, double h, const double* __re
       hi[f] = tmax(hi[f], x);
     }
     if constexpr (NC == 4) {
-      const double p = v[3] - fdiv(0.5 * (v[1] * v[1] + v[2] * v[2]), v[0]);
+      const double p = v[3] - sidp::fdiv(0.5 * (v[1] * v[1] + v[2] * v[2]), v[0]);
       if (p == p) pmin = tmin(pmin, p);
     }
   }
