@@ -387,13 +387,13 @@ cudaError_t run_steps(sidp_ctx* c, int nsteps) {
 // ---------------------------------------------------------------- tile autotuner
 // Picks the stage kernel's tile candidate per (law, p, precision, curved or not) by timing the launches of a
 // step (the time step, stage 1, and stage 2 twice: stage 3 would overwrite u^n, and moves the same data as stage
-// 2) with every candidate on the context's current state: node-layout tiles kTiles[p] and, for Euler,
-// line-layout tiles kLineTiles[p] (on a curved mesh: the node layout and the line layout).  Two
+// 2) with every candidate on the context's current state: node-layout tiles kTiles[p] but the small one and, for
+// Euler, line-layout tiles kLineTiles[p] (on a curved mesh: the node layout and the line layout).  Two
 // passes: at the first step, and once more at kSettleSteps steps, whose choice is kept for the
 // process.  Results differ between the layouts only in the rounding of sums.  SIDP_TILE=<i>
 // forces a candidate, SIDP_AUTOTUNE=0 keeps the default; SIDP_TUNE_FILE=<path> loads and stores
 // the settled table ("law p slot tile" lines, slot = precision (0 float64, 1 mixed) + 2 on a
-// curved mesh).
+// curved mesh; a line that names index 3, which older builds timed as a large tile, is passed over).
 std::mutex g_tune_mu;
 // last index: precision (0 float64, 1 mixed) + 2 on curved meshes
 int g_tune[LAW_ADVECTION_VAR + 1][kMaxP + 1][4];
@@ -414,7 +414,7 @@ void tune_table_init() {
       int law, p, mixed, tile;
       while (std::fscanf(fp, "%d %d %d %d", &law, &p, &mixed, &tile) == 4)
         if (law >= 1 && law <= 3 && p >= 1 && p <= kMaxP && mixed >= 0 && mixed <= 3 && tile >= 0 &&
-            tile < num_tile_candidates(law)) {
+            tile < num_tile_candidates(law) && tile != kSmallTile) {
           g_tune[law][p][mixed] = tile;
           g_settled[law][p][mixed] = true;
         }
@@ -489,14 +489,15 @@ cudaError_t autotune(sidp_ctx* c, bool second = false) {
   float best = 1e30f;
   int best_t = 0;
   const int saved = c->tile;
-  // candidates: every tile of both layouts on a Cartesian mesh; on a curved mesh the node layout
+  // candidates: the tiles of both layouts on a Cartesian mesh; on a curved mesh the node layout
   // (0) and, for Euler, the line layout (kNumTiles)
   int cand[kMaxCand], ncand = 0;
   if (c->curved) {
     cand[ncand++] = 0;
     if (c->cfg.law == LAW_EULER) cand[ncand++] = kNumTiles;
   } else {
-    for (int t = 0; t < num_tile_candidates(c->cfg.law); ++t) cand[ncand++] = t;
+    for (int t = 0; t < num_tile_candidates(c->cfg.law); ++t)
+      if (t != kSmallTile) cand[ncand++] = t;  // chosen by size only: the choice here serves meshes of every larger size
   }
   for (int ci = 0; ci < ncand && err == cudaSuccess; ++ci) {
     const int t = cand[ci];

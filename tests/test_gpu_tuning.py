@@ -1,0 +1,43 @@
+"""Which tile a context runs: the small one by size alone, the default one when tuning is off, and statistics that the
+tuner leaves alone."""
+import json
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+from paper_2004_08503_gb300 import inputs, sidp
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _child(code, **env):
+    """The tuner's table lives as long as the process: a fresh one per case."""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env={**os.environ, **env}, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    return json.loads(r.stdout.strip().splitlines()[-1])
+
+
+def test_a_stored_choice_of_the_small_tile_is_passed_over(tmp_path):
+    """Index 3 in a tuning file (older builds: a large tile) does not put a mesh of 256 default tiles on the
+    small one; the file's other lines hold, and the file that is written back names no 3."""
+    f = tmp_path / "tune"
+    f.write_text("2 3 1 3\n2 4 1 2\n")
+    code = """
+import json
+from paper_2004_08503_gb300 import inputs, sidp
+out = []
+for p in (3, 4):
+    sv = sidp.Solver(law="euler", p=p, nx=64, ny=64, precision="mixed", bc=("outflow",) * 4)
+    sv.set_state(inputs.four_quadrant(*sv.node_coords(), 0))
+    sv.set_stats(False)
+    sv.step(12)
+    out.append(sv.tile()[2])
+print(json.dumps(out))
+"""
+    tiles = _child(code, SIDP_TUNE_FILE=str(f))
+    assert tiles[0] != 3 and tiles[1] == 2
+    assert all(line.split()[3] != "3" for line in f.read_text().splitlines())
