@@ -461,17 +461,18 @@ cudaError_t autotune(sidp_ctx* c, bool second = false) {
   if (c->tuned && !second) return cudaSuccess;
   c->tuned = true;
   c->settle = false;
+  const char* off = std::getenv("SIDP_AUTOTUNE");
+  const bool keep = off && off[0] == '0', small = !keep && !c->curved && small_mesh(c->cfg);  // by size, not timed
   // only subcell limiting without the smoothness indicator has a stage kernel for every shape;
-  // the other modes run the default one
-  if (c->cfg.limiter != 2 || c->cfg.smoothness) { c->tile = (!c->curved && small_mesh(c->cfg)) ? kSmallTile : 0; return cudaSuccess; }
+  // the other modes run the default one or the small one
+  if (c->cfg.limiter != 2 || c->cfg.smoothness) { c->tile = small ? kSmallTile : 0; return cudaSuccess; }
   if (const char* f = std::getenv("SIDP_TILE")) {
     const int t = std::atoi(f);
     if (t >= 0 && t < num_tile_candidates(c->cfg.law)) c->tile = t;
     return cudaSuccess;
   }
-  const char* off = std::getenv("SIDP_AUTOTUNE");
-  if (off && off[0] == '0') return cudaSuccess;
-  if (!c->curved && small_mesh(c->cfg)) { c->tile = kSmallTile; return cudaSuccess; }  // by size, not timed
+  if (keep) return cudaSuccess;
+  if (small) { c->tile = kSmallTile; return cudaSuccess; }
   std::lock_guard<std::mutex> lk(g_tune_mu);
   tune_table_init();
   const int ti = (c->mixed ? 1 : 0) + (c->curved ? 2 : 0);

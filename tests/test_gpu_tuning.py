@@ -41,3 +41,15 @@ print(json.dumps(out))
     tiles = _child(code, SIDP_TUNE_FILE=str(f))
     assert tiles[0] != 3 and tiles[1] == 2
     assert all(line.split()[3] != "3" for line in f.read_text().splitlines())
+
+
+@pytest.mark.parametrize("cfg", [dict(limiter="none"), dict(limiter="lo"), dict(limiter="subcell"), dict(limiter="elementwise"),
+                                 dict(limiter="subcell", smoothness=dict(gmin=-0.5, gmax=1.6))])
+def test_no_tuning_keeps_the_default_tile_in_every_mode(cfg, monkeypatch):
+    for off in (True, False):
+        monkeypatch.setenv("SIDP_AUTOTUNE", "0" if off else "1")
+        sv = sidp.Solver(law="euler", p=3, nx=6, ny=6, bc=("outflow",) * 4, **cfg)
+        sv.set_state(inputs.four_quadrant(*sv.node_coords(), 0))
+        sv.step(1)
+        assert sv.tile()[2] == (0 if off or cfg["limiter"] == "elementwise" else 3)
+        sv.close()
