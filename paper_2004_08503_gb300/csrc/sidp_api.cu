@@ -483,8 +483,12 @@ cudaError_t autotune(sidp_ctx* c, bool second = false) {
     if (!settled) { c->settle = true; c->settle_at = c->steps + kSettleSteps; }
     return cudaSuccess;
   }
+  // the timed launches run the statistics kernels when those are on: what they count is not the run's
+  StageStats stats;
+  cudaError_t err = cudaMemcpyAsync(&stats, c->d_stats, sizeof(stats), cudaMemcpyDeviceToHost, c->stream);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(c->stream);
   cudaEvent_t e0, e1;
-  cudaError_t err = cudaEventCreate(&e0);
+  if (err == cudaSuccess) err = cudaEventCreate(&e0);
   if (err != cudaSuccess) return err;
   if ((err = cudaEventCreate(&e1)) != cudaSuccess) { cudaEventDestroy(e0); return err; }
   float best = 1e30f;
@@ -520,6 +524,7 @@ cudaError_t autotune(sidp_ctx* c, bool second = false) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(c->d_stats, &stats, sizeof(stats), cudaMemcpyHostToDevice, c->stream);
   if (err != cudaSuccess) { c->tile = saved; return err; }
   c->tile = best_t;
   slot = best_t;

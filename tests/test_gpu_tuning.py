@@ -53,3 +53,32 @@ def test_no_tuning_keeps_the_default_tile_in_every_mode(cfg, monkeypatch):
         sv.step(1)
         assert sv.tile()[2] == (0 if off or cfg["limiter"] == "elementwise" else 3)
         sv.close()
+
+
+def test_the_statistics_are_the_runs_own():
+    """One step whose tile is chosen by timing reports what the same step reports on that tile without timing: the
+    candidates' launches leave no count and no maximum behind (every degree, so that each is timed once)."""
+    code = """
+import json
+from paper_2004_08503_gb300 import inputs, sidp
+keys = ("max_bound_violation", "max_entropy_violation", "rootfind_max_iters", "rootfind_cap_hits", "bound_nudges")
+out = []
+for prec in ("mixed", "fp64"):
+    for p, n in ((1, 200), (2, 120), (3, 80), (4, 60), (5, 50), (6, 48), (7, 48)):
+        runs, tile = [], None
+        for pin in (False, True):
+            sv = sidp.Solver(law="euler", p=p, nx=n, ny=n, precision=prec, bc=("outflow",) * 4)
+            sv.set_state(inputs.four_quadrant(*sv.node_coords(), 2))
+            if pin:
+                sv.set_tile(tile)
+            sv.step(1)
+            tile = sv.tile()[2]
+            d = sv.diag()
+            runs.append([d[k] for k in keys])
+            sv.close()
+        assert tile != 3
+        out.append([prec, p, runs])
+print(json.dumps(out))
+"""
+    for prec, p, (timed, pinned) in _child(code):
+        assert timed == pinned, (prec, p, timed, pinned)
