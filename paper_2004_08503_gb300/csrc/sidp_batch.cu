@@ -413,8 +413,12 @@ cudaError_t tune_batch(sidp_batch* b) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  if (e == cudaSuccess) e = cudaMemcpy(b->d_clock, clock.data(), b->n * sizeof(double), cudaMemcpyHostToDevice);
+  // arms the minima of the timed time-step launches again and puts the clocks back, after a failed pass too: the next
+  // step's time steps are its own
+  k_batch_finalize<<<(b->n + 127) / 128, 128, 0, b->stream>>>(b->d_bits, b->d_cfl, b->d_dt, b->d_dtf, b->d_clock, b->n);
+  for (cudaError_t e2 : {cudaGetLastError(), cudaStreamSynchronize(b->stream),
+                         cudaMemcpy(b->d_clock, clock.data(), b->n * sizeof(double), cudaMemcpyHostToDevice)})
+    if (e == cudaSuccess) e = e2;
   return e;
 }
 
