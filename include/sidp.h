@@ -142,7 +142,8 @@ sidp_status sidp_node_coords(const sidp_ctx* ctx, double* x, double* y);
 sidp_status sidp_set_state(sidp_ctx* ctx, const double* u);
 
 /* Copy a state out as float64 [nc][N].  which = 0: the current solution u^n; 1: the stage-1
- * result u^(1); 2: the stage-2 result u^(2) (SSP-RK3, Sec. 5).  Synchronises the stream. */
+ * result u^(1); 2: the stage-2 result u^(2) (SSP-RK3, Sec. 5).  Synchronises the stream.  SIDP_MIXED: read
+ * through 1 MiB of page-locked memory that the first call allocates and the context keeps. */
 sidp_status sidp_get_state(sidp_ctx* ctx, int which, double* u);
 
 /* Asynchronous state transfer in the library's storage type (float64 for SIDP_FP64, float32
@@ -247,20 +248,29 @@ sidp_status sidp_stage(sidp_ctx* ctx, int k, double dt);
 
 /* nsteps SSP-RK3 steps, each with dt from Eq. cfl-low evaluated on u^n (computed on the
  * device; no host synchronisation).  Asynchronous.  The first call captures one step as a
- * CUDA graph (when use_graph is on) and later calls replay it. */
+ * CUDA graph (when use_graph is on) and later calls replay it.  A Cartesian mesh of at most 16 small
+ * tiles (see sidp_get_tile) under subcell limiting without the smoothness indicator runs its steps inside one
+ * launch per 256 steps instead, a thread-block cluster with one CTA per tile, where the device can hold the
+ * cluster; no graph is made then. */
 sidp_status sidp_step(sidp_ctx* ctx, int nsteps);
 
-/* Element tile (elements per CTA along x and y) that the stage kernels use; chosen per
- * (law, p, precision, Cartesian or curved) by timing the candidates at the first sidp_step and once more when the
- * context has taken 10 steps (the first steps of a flow, such as a blast's initial transient,
- * can favour another tile than the rest of the run; that second pass synchronizes the stream
- * once, inside the sidp_step call that reaches step 10).  SIDP_TILE=<index> forces one,
- * SIDP_AUTOTUNE=0 keeps the default, SIDP_TUNE_FILE=<path> persists the settled choices.  The
- * candidates are indices 0..3, tiles of the node kernel (one thread per node), and, for the
- * Euler law, indices 4..5, tiles of the line kernel (one thread per element line).  Both compute
- * the same stage update (Sec. 4 with subcell limiting); they differ in the order of the rounding
- * of sums.  Modes other than subcell limiting without the smoothness indicator run the node
- * kernel with tile 0. */
+/* Element tile (elements per CTA along x and y) that the stage kernels use.  Candidates: indices 0..3, tiles of
+ * the node kernel (one thread per node), of which 0 is the default and 3 the small one (one or two
+ * warps per CTA), and, for the Euler law, indices 4..5, tiles of the line kernel (one thread per element
+ * line).  All compute the same stage update (Sec. 4 with subcell limiting); they differ in the order of the
+ * rounding of sums.
+ *   Small Cartesian meshes take index 3 at the first sidp_step, by their size and in every mode but elementwise
+ * limiting and the unsparsified operator: up to 200 default tiles in SIDP_FP64, up to 100 in SIDP_MIXED and
+ * for the unlimited scheme.
+ *   Larger ones, under subcell limiting without the smoothness indicator: chosen per (law, p, precision,
+ * Cartesian or curved) by timing the candidates but the small one at the first sidp_step and once more when
+ * the context has taken 10 steps (the first steps of a flow, such as a blast's initial transient, can favour
+ * another tile than the rest of the run; that second pass synchronizes the stream once, inside the
+ * sidp_step call that reaches step 10).  The timing leaves state, clock and statistics as they are.
+ *   Other modes: index 0.
+ * SIDP_TILE=<index> forces a candidate for subcell limiting without the indicator, SIDP_AUTOTUNE=0 keeps
+ * index 0 in every mode, SIDP_TUNE_FILE=<path> persists the settled choices of the timing (a line that names
+ * index 3 is passed over). */
 sidp_status sidp_get_tile(const sidp_ctx* ctx, int* tx, int* ty);
 
 /* The candidate index of the tile in use (see sidp_get_tile): 0..3 node kernel, 4..5 line
@@ -269,19 +279,21 @@ sidp_status sidp_get_tile_index(const sidp_ctx* ctx, int* index);
 
 /* Use tile candidate `index` (see sidp_get_tile) from now on, instead of the autotuner's choice.
  * Index 0 is valid in every mode; the others only for subcell limiting without the smoothness
- * indicator and the unsparsified mode: on a Cartesian mesh 1..3 (node kernel) and, for the Euler
+ * indicator and the unsparsified mode: on a Cartesian mesh 1..3 (node kernel; 3 is the small tile) and, for the Euler
  * law, 4..5 (line kernel); on a curved mesh (after sidp_set_geometry) 4, the curved line kernel,
  * for the Euler law.  Otherwise SIDP_ERR_ARG.  SIDP_ERR_STATE between stages 1 and 3 of an
  * explicit step.  sidp_set_geometry returns a context to tile 0 and to autotuning. */
 sidp_status sidp_set_tile(sidp_ctx* ctx, int index);
 
-/* Enable (1) or disable (0) CUDA-graph replay in sidp_step (default 1). */
+/* Enable (1) or disable (0) CUDA-graph replay in sidp_step (default 1).  Without effect where sidp_step runs whole
+ * steps in one launch. */
 sidp_status sidp_set_graph(sidp_ctx* ctx, int use_graph);
 
 /* Enable (1) / disable (0) the per-stage statistics reported in sidp_diag, on by default: bound
  * and entropy violations and root-search counters.  With them on, a statistics variant of the stage kernel
- * runs (default tile shape); in the float32 form it evaluates the entropy bound accurately and
- * costs about 2.5x a plain stage.  Turn them off for timed runs. */
+ * runs (the default, the small or the line kernel's tile; indices 1 and 2 run it on the default one); in the float32
+ * form it evaluates the entropy bound accurately at the nodes where a cheap test leaves it open and costs about
+ * 1.3x a plain stage.  Turn them off for timed runs. */
 sidp_status sidp_set_stats(sidp_ctx* ctx, int on);
 
 /* Debug capture: when on, every later stage writes its local bounds (lo, hi of the limited field;
