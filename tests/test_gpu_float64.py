@@ -1,5 +1,5 @@
 """The float64 path where its cheap forms meet their limits: densities far from 1, nodes
-without a real sound speed."""
+without a real sound speed, infinite values under the smoothness indicator."""
 import numpy as np
 import pytest
 
@@ -51,3 +51,30 @@ def test_negative_pressure_at_a_face_keeps_the_neighbours_speed(node, limiter, p
     got = sv.get_state(1)
     sv.close()
     assert np.all(np.isfinite(got))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("curved", [False, True])
+def test_an_infinite_indicator_allows_no_flux(curved, precision):
+    """An element with an infinite density has no indicator (infinity over infinity) and NaN bounds, which
+    allow no antidiffusive flux: its nodes off the infinite one's lines take the low-order update, to 1e-12 of the
+    state's size (float32: 2e-5)."""
+    got = []
+    for cfg in (dict(limiter="subcell", smoothness=dict(gmin=-0.5, gmax=2.5)), dict(limiter="lo")):
+        sv = sidp.Solver(law="advection", p=3, nx=7, ny=6, domain=(0.0, 1.4, 0.0, 1.2), bc=("periodic",) * 4, beta=(0.7, -0.4),
+                         precision=precision, **cfg)
+        x, y = sv.node_coords()
+        if curved:
+            b = 0.02 * np.sin(2 * np.pi * x / 1.4) * np.sin(2 * np.pi * y / 1.2)
+            sv.set_geometry(x + b, y + b)
+        u = 1.0 + np.sin(9 * x) * np.cos(8 * y)
+        base = (2 * 7 + 3) * 16
+        u[base + 5] = np.inf
+        v = np.ascontiguousarray(u[None], dtype=np.float64 if precision == "fp64" else np.float32)
+        sidp.sidp_upload_state(sv.ctx, v.ctypes.data)
+        sv.stage(1, 2e-3)
+        got.append(sv.get_state(1)[0, base:base + 16].reshape(4, 4))
+        sv.close()
+    off = np.ix_([0, 2, 3], [0, 2, 3])
+    a, b = got[0][off], got[1][off]
+    assert np.all(np.isfinite(b)) and np.max(np.abs(a - b)) <= (1e-12 if precision == "fp64" else 2e-5) * 2.0
