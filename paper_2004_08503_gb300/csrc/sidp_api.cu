@@ -85,7 +85,7 @@ __device__ __forceinline__ void diag_reduce(double* acc, double (*red)[kDiagThre
 
 // Diagnostics of a state in one launch: every block's sums and extremes into `part`, the last block's
 // reduction of them with the clock and the statistics into `out`.  The extremes are taken in the stored
-// type and the masses of a node from a table, so that a node costs 14 float64 operations (its products
+// type and the masses of a node from a table, so that a node costs 13 float64 operations (its products
 // with the mass, its pressure); 60 with float64 minima, products of weights and an IEEE division, and one
 // thread reducing the blocks, took 258 us on any small mesh and 1.9 ms on 16.8M nodes.
 template <typename T, int NC>
