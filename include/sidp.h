@@ -260,8 +260,8 @@ sidp_status sidp_step(sidp_ctx* ctx, int nsteps);
  * line).  All compute the same stage update (Sec. 4 with subcell limiting); they differ in the order of the
  * rounding of sums.
  *   Small Cartesian meshes take index 3 at the first sidp_step, by their size and in every mode but elementwise
- * limiting and the unsparsified operator: up to 200 default tiles in SIDP_FP64, up to 100 in SIDP_MIXED and
- * for the unlimited scheme.
+ * limiting and the unsparsified operator: up to 200 default tiles in SIDP_FP64 under subcell limiting, 81 for
+ * its unlimited and low-order schemes, 100 in SIDP_MIXED.
  *   Larger ones, under subcell limiting without the smoothness indicator: chosen per (law, p, precision,
  * Cartesian or curved) by timing the candidates but the small one at the first sidp_step and once more when
  * the context has taken 10 steps (the first steps of a flow, such as a blast's initial transient, can favour

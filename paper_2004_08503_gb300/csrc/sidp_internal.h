@@ -78,16 +78,19 @@ constexpr TileShape kTiles[kMaxP + 1][kNumTiles] = {
     {{1, 5}, {5, 1}, {2, 2}, {1, 1}},    // p=6: 245 / 245 / 196 / 49
     {{1, 4}, {4, 1}, {2, 2}, {1, 1}},    // p=7: 256 / 256 / 256 / 64
 };
-// A Cartesian mesh of up to so many default tiles takes the small tile.  float64: a step took (us, default / small
-// tile) 169 / 147 at 100 tiles, 171 / 169 at 121, 250 / 230 at 196 and 251 / 270 at 256 (Euler p = 3), 179 / 153 at
-// 96, 266 / 227 at 160 and 269 / 277 at 216 (p = 5), 41 / 37 at 100 and 62 / 54 at 196 (Burgers p = 3): an SM's
-// two float64 lanes are what the warps of its CTAs share.  float32 (latency alone): equal within 2 us at every
-// size up to 256 tiles; 100 keeps the timed candidates for larger meshes.  The unlimited scheme, whose kernel is
-// mostly halo on a small tile, took 43 / 49 us a step at 112 tiles (float64, p = 4).
+// A Cartesian mesh of up to so many default tiles takes the small tile: an SM's two float64 lanes are what the warps
+// of its CTAs share.  float64, us a step (default / small tile).  Subcell limiting, 200: Euler p = 3 169 / 147 at
+// 100 tiles, 171 / 169 at 121, 250 / 230 at 196 and 251 / 270 at 256; p = 5 179 / 153 at 96, 266 / 227 at 160
+// and 269 / 277 at 216; p = 3 with the indicator or without, at 196: Burgers 82 / 68 and 68 / 57, advection 80 / 68
+// and 66 / 55, varying velocity 90 / 74 and 76 / 64.  Unlimited and low-order schemes, 81: a halo is more of their work;
+// Euler p = 1..7 at 81 tiles 70..74 / 61..62 and 111..123 / 94..102, at 100 from 70 / 61 (p = 3) to 72 / 78
+// (p = 5) and from 113 / 102 (p = 7) to 121 / 135 (p = 5).  float32 (latency alone): equal within 2 us at every
+// size up to 256 tiles; 100 keeps the timed candidates for larger meshes.
 inline bool small_mesh(const sidp_config& c) {
   const TileShape t = kTiles[c.p][0];
   const long long ctas = (long long)((c.nx + t.tx - 1) / t.tx) * ((c.ny + t.ty - 1) / t.ty);
-  return c.limiter != SIDP_LIMITER_ELEMENTWISE && !c.unsparsified && ctas <= (c.precision == SIDP_FP64 && c.limiter != SIDP_LIMITER_NONE ? 200 : 100);
+  const int limit = c.precision != SIDP_FP64 ? 100 : c.limiter == SIDP_LIMITER_SUBCELL ? 200 : 81;
+  return c.limiter != SIDP_LIMITER_ELEMENTWISE && !c.unsparsified && ctas <= limit;
 }
 
 // Element tiles of the line-parallel stage kernel (one thread per element line; Euler, subcell

@@ -82,3 +82,19 @@ print(json.dumps(out))
 """
     for prec, p, (timed, pinned) in _child(code):
         assert timed == pinned, (prec, p, timed, pinned)
+
+
+@pytest.mark.parametrize("limiter,precision,tiles,small", [
+    ("none", "fp64", (9, 9), True), ("none", "fp64", (9, 10), False), ("lo", "fp64", (9, 9), True), ("lo", "fp64", (10, 9), False),
+    ("subcell", "fp64", (10, 20), True), ("subcell", "fp64", (11, 19), False), ("none", "mixed", (10, 10), True),
+    ("subcell", "mixed", (10, 10), True), ("subcell", "mixed", (10, 11), False)])
+def test_the_size_rule_of_the_small_tile(limiter, precision, tiles, small):
+    """Meshes on each side of the rule's line (p = 3: default tiles of 4 x 4 elements)."""
+    nx, ny = 4 * tiles[0], 4 * tiles[1]
+    sv = sidp.Solver(law="euler", p=3, nx=nx, ny=ny, domain=(0.0, 1.0, 0.0, ny / nx), bc=("outflow",) * 4, limiter=limiter,
+                     precision=precision)
+    sv.set_state(inputs.four_quadrant(*sv.node_coords(), 0) if limiter != "none" else
+                 np.repeat(inputs._cons(np.array([1.0]), np.array([0.1]), np.array([0.0]), np.array([1.0])), sv.N, axis=1))
+    sv.step(1)
+    assert (sv.tile()[2] == 3) == small
+    sv.close()
