@@ -48,11 +48,11 @@ STAGE_COUNTERS = {
     # active 36.5% of the cycles of stage 2 in the capture
     "line": {"kernel": "k_stage_lines<3, TX, TY, LawEuler<float>, float>", "current": True,
              "dram_bytes_per_node": 38.7, "fp32_flop_per_node": None,
-             "warp_instr_per_node": (15.81, 15.81, 15.81)},
+             "warp_instr_per_node": (15.82, 15.82, 15.82)},
 }
 # The float64 stage kernel's executed FP64 flops per node (2 x DFMA + DADD + DMUL), stages 1-3,
 # from an ncu capture of the same workload in float64 (the line kernel, 8x4 tile): its FP64-pipe roofline.
-FP64_STAGE_FLOP_PER_NODE = (500.8, 512.8, 512.8)
+FP64_STAGE_FLOP_PER_NODE = (575.3, 587.3, 587.3)
 SMS, SCHEDULERS_PER_SM = 152, 4
 # DRAM traffic per node and launch (stages 1-3 averaged) of the two curved-mesh stage kernels, from
 # ncu captures of the 768x768 curved leg; "current" is False once the kernel has changed since.
